@@ -1,6 +1,6 @@
 """The Grams of the option fp64_tc above width 8 (tcgen05, exact digits) at the edges of their 64-bit frame: a
 128-row tile whose columns are constant just below a power of two, where the sum of a digit stack comes close to
-the frame's end.
+the frame's end; and the diagonal of an unconjugated Gram, sum re^2 - sum im^2, where the two nearly cancel.
 
 Bounds: the factor xi_0 of the residual's Cholesky QR satisfies xi^H xi = R^H R; with unit-variance rows the Gram
 and its Cholesky factor are accurate to a few hundred roundings (p n-term sums, condition below 10): 1e-12 of the
@@ -55,3 +55,48 @@ def test_constant_columns_near_full_scale(method, p, imag):
         assert h.solve(B, X, method=method, tol=0.0, maxit=1) == blcoc.BLCOC_NOT_CONVERGED
     f = O.bl_cocr_rq if method == "cocr_rq" else O.bl_cocg_rq
     assert rel(X.cpu().numpy(), f(A, Bh, tol=0.0, maxit=1).X) < 1e-10
+
+
+def _cancelling(n, p, method, seed):
+    """Columns of disjoint support whose Gram V^T V (bl_cocg_rq) or V^T A V (bl_cocr_rq), A diagonal, has diagonal
+    entries of about 0.02 although sum re^2 and sum im^2 are in the thousands; entries of 30 bits, so that every sum up
+    to re - im is exact.  The other Gram that the first iterate depends on, V^T A V or V^T A^2 V, does not cancel.
+    Returns the rows' values, A's diagonal, the columns and the exact diagonals of both."""
+    rng = np.random.default_rng(seed)
+    m = n // 2
+    k = rng.integers(2**28, 2**30, m)
+    cocg = method == "cocg_rq"
+    k2 = np.minimum(np.rint(k * (1 + 1e-3 * rng.standard_normal(m)) / (1 if cocg else np.sqrt(2))), 2.0**30 - 1)
+    z, a = np.empty(n, np.complex128), np.empty(n, np.complex128)
+    z[0::2], z[1::2] = k, (1j if cocg else 1 + 1j) * k2
+    a[0::2], a[1::2] = 1, -1 if cocg else 1j
+    col = np.arange(m) % p
+    k2 = k2.astype(np.int64)
+    G, H = np.empty(p), np.empty(p, np.complex128)
+    for j in range(p):
+        x, y = (sum(int(v) ** 2 for v in w[col == j]) for w in (k, k2))
+        G[j] = (x - (y if cocg else 2 * y)) / 2**60
+        H[j] = (x + y) / 2**60 if cocg else complex(x / 2**60, -2 * y / 2**60)
+    return z * 2.0**-30, a, np.repeat(col, 2), G, H
+
+
+@pytest.mark.parametrize("p", [9, 17, 32])
+@pytest.mark.parametrize("method", ["cocg_rq", "cocr_rq"])
+def test_diagonal_of_an_unconjugated_gram_keeps_its_small_part(method, p):
+    """X_1 = V diag(G / H): the error of G's diagonal is read off X_1 (G is small, so that all other roundings are, too:
+    some 1e-16 of 0.02).  Bound 2e-15 rms over the columns: each of at most 304 CTAs rounds four differences of its
+    stacks, below 0.1, i.e. sqrt(304 * 4) * 0.1 * 2^-54 = 2e-16 rms, with a factor of ten.  Sums rounded before the
+    difference miss it by a factor of five: emulated, 1.4e-14."""
+    torch = need_gpu()
+    from paper_1601_05362_gb300 import blcoc
+    n = 200064
+    z, a, col, G, H = _cancelling(n, p, method, seed=p)
+    Bh = np.zeros((n, p), np.complex128)
+    Bh[np.arange(n), col] = z
+    with blcoc.Handle(n, np.arange(n + 1, dtype=np.int32), np.arange(n, dtype=np.int32), a) as h:
+        h.set_option("fp64_tc", 1)
+        B = to_dev(torch, Bh)
+        X = torch.zeros_like(B)
+        assert h.solve(B, X, method=method, tol=0.0, maxit=1) == blcoc.BLCOC_NOT_CONVERGED
+        M = (torch.sum(B.conj() * X, 0) / torch.sum(B.abs().square(), 0)).cpu().numpy()
+    assert np.sqrt(np.mean(np.abs(M * H - G) ** 2)) < 2e-15
