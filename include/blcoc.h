@@ -44,7 +44,7 @@ typedef enum {
   BLCOC_NOT_CONVERGED = 5,     /* maxit iterations ran without reaching tol              */
   BLCOC_BREAKDOWN = 6,         /* the residual block lost rank, a p x p system was
                                   singular, or a coefficient became non-finite          */
-  BLCOC_ERR_TIMEOUT = 7        /* reserved: a device wait gave up                        */
+  BLCOC_ERR_TIMEOUT = 7        /* a wait inside a kernel gave up; X is unfinished        */
 } blcoc_status;
 
 /* Methods.  The _MIXED forms are iterative refinement around the rq methods: the residual
@@ -277,6 +277,10 @@ blcoc_status blcoc_sampled_grad(blcoc_handle h, const void* Lambda, const void* 
  *   "persistent_stall": blcoc_solve_batched_persistent (read from hs[0]), a test of the
  *                  time limit: 1 publishes no first work item, so every wait for work
  *                  runs out and the call returns BLCOC_ERR_TIMEOUT (0 = off, default).
+ *   "lost_wait"  : a test of the same report by the other solves: 1 lets the next solve on
+ *                  this handle end as if a kernel of it had given up a wait (it returns
+ *                  BLCOC_ERR_TIMEOUT and leaves the reductions' arrival counters as such a
+ *                  kernel may), and is 0 again after it (0 = off, default).
  *   "timing"     : 1 brackets every kernel of the iterations with CUDA events on
  *                  the internal stream (also inside the graph) and accumulates per-kernel
  *                  device time; 2 brackets only the row-pass kernels (less overhead:

@@ -147,6 +147,7 @@ struct blcoc_ctx {
   Ctrl* ctrl = nullptr;
   Ctrl* h_ctrl = nullptr;    // pinned
   unsigned* slice_cnt = nullptr;   // arrival counters of the reductions fused into the passes (behind flags)
+  bool counting = false;           // a call that uses them has begun and not ended in order, see begin_counting
   int* flags = nullptr;
   // options
   int use_graph = 1;
@@ -172,6 +173,7 @@ struct blcoc_ctx {
   int stat_spmm_split = 0;    // row bundle of the last solve
   int persistent_timeout_ms = 10000;   // persistent batch: limit of one wait of the kernel
   int persistent_stall = 0;   // persistent batch, test hook: no first work item is published
+  int lost_wait = 0;          // test hook: the next solve ends as if a kernel's wait had run out
   int stat_persistent_graph = -1;   // last persistent batch: 1 graph replays, 0 direct launches
   Graph graph;      // iterations without the QR fallback's launches
   Graph graph_fb;   // iterations with them, used once a solve has needed the fallback
@@ -273,6 +275,30 @@ blcoc_status ensure_ws(blcoc_ctx* h, int p) {
   h->p_cap = p;
   h->gen++;
   return BLCOC_OK;
+}
+
+// Every call whose passes count arrivals begins here, on the handle's stream, and ends with end_counting.  One that
+// did not end in order (an error return, a kernel whose wait ran out) may have left CTAs uncounted; a later
+// reduction would then add up partial sums that are not written yet.
+blcoc_status begin_counting(blcoc_ctx* h) {
+  if (h->counting) CK(h, cudaMemsetAsync(h->slice_cnt, 0, (RED_SPLIT + 1) * sizeof(unsigned), h->s));
+  h->counting = true;
+  return BLCOC_OK;
+}
+// c: the control block the call ended with.  False (and the handle's message) if a kernel's wait had run out.
+bool end_counting(blcoc_ctx* h, Ctrl& c) {
+  if (h->lost_wait) {   // the test hook leaves what such a kernel does: a count too many in every slice
+    h->lost_wait = 0;
+    c.done = 3;
+    c.bd_code = BD_WAIT;
+    cudaMemsetAsync(h->slice_cnt, 1, (RED_SPLIT + 1) * sizeof(unsigned), h->s);
+  }
+  if (c.done == 3 && c.bd_code == BD_WAIT) {
+    h->err = "a wait inside a kernel ran out; X holds an unfinished iterate";
+    return false;
+  }
+  h->counting = false;
+  return true;
 }
 
 }  // namespace
@@ -917,6 +943,11 @@ blcoc_status blcoc_set_option(blcoc_handle h, const char* key, int64_t value) {
     h->persistent_stall = (int)value;
     return BLCOC_OK;
   }
+  if (!strcmp(key, "lost_wait")) {
+    if (value != 0 && value != 1) return invalid(h, "lost_wait must be 0 or 1");
+    h->lost_wait = (int)value;
+    return BLCOC_OK;
+  }
   return invalid(h, "unknown option");
 }
 
@@ -972,10 +1003,13 @@ blcoc_status blcoc_residual_norm(blcoc_handle h, const void* B, const void* X, i
   sv.K->prepare();
   CK(h, cudaEventRecord(h->ev, h->user_stream));
   CK(h, cudaStreamWaitEvent(h->s, h->ev, 0));
+  st = begin_counting(h);
+  if (st != BLCOC_OK) return st;
   sv.true_residual();
   CK(h, cudaGetLastError());
   CK(h, cudaMemcpyAsync(h->h_ctrl, h->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->s));
   CK(h, cudaStreamSynchronize(h->s));
+  h->counting = false;
   *out = h->h_ctrl->trr;
   return BLCOC_OK;
 }
@@ -1185,8 +1219,11 @@ blcoc_status solve_mixed(blcoc_ctx* h, const double2* dB, double2* dX, void* X, 
   h->relres = relres;
   h->hist_h = outer_hist;
   h->xi_h.assign(2 * p * p, 0.0);
+  Ctrl last = *h->h_ctrl;
+  const bool in_order = end_counting(h, last);
   st = finish_solve(h, sv, X, hostX, bytes);
   if (st != BLCOC_OK) return st;
+  if (!in_order) return BLCOC_ERR_TIMEOUT;
   switch (done) {
     case 1: return BLCOC_OK;
     case 2: return BLCOC_NOT_CONVERGED;
@@ -1501,6 +1538,8 @@ blcoc_status blcoc_solve(blcoc_handle h, const void* B, void* X, int p, blcoc_me
   }
   CK(h, cudaEventRecord(h->ev, h->user_stream));
   CK(h, cudaStreamWaitEvent(h->s, h->ev, 0));
+  st = begin_counting(h);
+  if (st != BLCOC_OK) return st;
   const double2* dB = (const double2*)B;
   double2* dX = (double2*)X;
   if (hostB) {
@@ -1532,8 +1571,6 @@ blcoc_status blcoc_solve(blcoc_handle h, const void* B, void* X, int p, blcoc_me
     sv.oz = h->ozbuf;
   }
   sv.K->prepare();
-  if (h->h_ctrl->bd_code == 7)   // a kernel's wait had run out: some of its CTAs may not have been counted
-    CK(h, cudaMemsetAsync(h->slice_cnt, 0, (RED_SPLIT + 1) * sizeof(unsigned), h->s));
   sv.use_fp64_blocks();
   sv.spmm_two = true;
   sv.plain = plain ? 1 : 0;
@@ -1589,7 +1626,8 @@ blcoc_status blcoc_solve(blcoc_handle h, const void* B, void* X, int p, blcoc_me
   CK(h, cudaGetLastError());
   CK(h, cudaMemcpyAsync(h->h_ctrl, h->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->s));
   CK(h, cudaStreamSynchronize(h->s));
-  const Ctrl c = *h->h_ctrl;
+  Ctrl c = *h->h_ctrl;
+  const bool in_order = end_counting(h, c);
   h->iters = zero_rhs ? 0 : c.iter;
   const double nb = std::sqrt(c.sumsq_b);
   h->trr = zero_rhs ? 0.0 : (nb > 0 ? c.trr / nb : NAN);
@@ -1604,6 +1642,7 @@ blcoc_status blcoc_solve(blcoc_handle h, const void* B, void* X, int p, blcoc_me
                    cudaMemcpyDeviceToHost));
   st = finish_solve(h, sv, X, hostX, bytes);
   if (st != BLCOC_OK) return st;
+  if (!in_order) return BLCOC_ERR_TIMEOUT;
   if (zero_rhs) return BLCOC_OK;
   switch (c.done) {
     case 1: return BLCOC_OK;
@@ -1658,6 +1697,8 @@ static blcoc_status solve_batched_impl(int form, int nsys, const blcoc_handle* h
     }
     CK(h, cudaEventRecord(h->ev, h->user_stream));
     CK(h, cudaStreamWaitEvent(h->s, h->ev, 0));
+    st = begin_counting(h);
+    if (st != BLCOC_OK) return st;
     int PP = 0;
     sv.push_back(Solver{h, kernels_for(p[i], &PP), PP, p[i], (int)method, (const double2*)B[i], (double2*)X[i]});
     // per-system options, as in blcoc_solve: tensor-core block updates, explicit U, CholQR2
@@ -1868,7 +1909,8 @@ static blcoc_status solve_batched_impl(int form, int nsys, const blcoc_handle* h
     s1.true_residual();
     CK(h, cudaMemcpyAsync(h->h_ctrl, h->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->s));
     CK(h, cudaStreamSynchronize(h->s));
-    const Ctrl c = *h->h_ctrl;
+    Ctrl c = *h->h_ctrl;
+    const bool in_order = end_counting(h, c);
     h->iters = c.iter;
     const double nb = std::sqrt(c.sumsq_b);
     h->trr = nb > 0 ? c.trr / nb : 0.0;
@@ -1881,6 +1923,7 @@ static blcoc_status solve_batched_impl(int form, int nsys, const blcoc_handle* h
     CK(h, cudaStreamWaitEvent(h->user_stream, h->ev, 0));
     h->stat_launches = launches;
     blcoc_status si = c.done == 1 || nb == 0 ? BLCOC_OK : (c.done == 2 ? BLCOC_NOT_CONVERGED : BLCOC_BREAKDOWN);
+    if (!in_order) worst = BLCOC_ERR_TIMEOUT;
     if (si != BLCOC_OK && worst == BLCOC_OK) worst = si;
   }
   if (!shape_msg.empty() && worst == BLCOC_OK && h0) h0->err = shape_msg;

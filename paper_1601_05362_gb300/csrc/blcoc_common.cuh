@@ -25,6 +25,8 @@ constexpr int SMALL_THREADS = 256;
 #define BLCOC_LD(ptr) (*(ptr))
 #endif
 
+constexpr int BD_WAIT = 7;      // Ctrl::bd_code of a solve whose kernel gave up a wait
+
 // Device-resident control block of one solve.  Kernels of an iteration return at once
 // when `done` is non-zero, so a batch of queued iterations past convergence is a no-op.
 struct Ctrl {
@@ -33,7 +35,8 @@ struct Ctrl {
                   // before the Cholesky QR (a pass's own stage could not complete it)
   int iter;       // m: X holds X_m
   int maxit;
-  int bd_code;    // breakdown site: 1 setup QR, 2 alpha solve, 3 QR, 4 beta solve, 5 non-finite xi
+  int bd_code;    // breakdown site: 1 setup QR, 2 alpha solve, 3 QR, 4 beta solve, 5 non-finite xi,
+                  // BD_WAIT: no breakdown, a wait inside a kernel ran out
   int nhist;      // entries of the residual history written so far
   int hlu_ok;     // cocr: the LU factors of H_m in slots M_HLU (beside the alpha' step) are valid
   int qr_fb;      // shifted-CholQR3 fallback: re-orthogonalising passes still to run (0: none)
