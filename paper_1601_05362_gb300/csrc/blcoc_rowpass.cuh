@@ -1567,13 +1567,14 @@ __global__ void __launch_bounds__(256) k_axpy(const PassArgs a) {
 // First-stage reduction of a pass's Gram partials inside the pass (a.slice_cnt set): of the CTAs
 // of a slice the one that arrives last sums the slice's partials, in k_reduce_stage1's order,
 // so the sums are the same bits.  Saves that kernel's launch (about 3.5 us of a 2D iteration)
-// where one CTA can sum a slice as quickly: see Solver::fused_reduce for the line.
+// where one CTA can sum a slice as quickly: see Solver::fuse_reduce for the line.
 // Returns whether this CTA summed the last slice of all (with a.tail; its slices are then all written).
 __device__ __forceinline__ bool slice_reduce(const PassArgs& a) {
   if (a.slice_cnt == nullptr) return false;
-  if (!(a.flag & F_FORCE) && BLCOC_LD(&a.ctrl->done)) return false;
-  if ((a.flag & F_FB) && BLCOC_LD(&a.ctrl->qr_fb) == 0) return false;
   __shared__ int last;
+  // one read for the CTA: a tcgen05 kernel's CTA that gave up a wait sets `done` while others are here
+  const bool off = threadIdx.x == 0 && ((!(a.flag & F_FORCE) && BLCOC_LD(&a.ctrl->done)) ||
+                                        ((a.flag & F_FB) && BLCOC_LD(&a.ctrl->qr_fb) == 0));
   const int G = gridDim.x, q = blockIdx.x;
   int s = (int)((int64_t)q * RED_SPLIT / G);
   while ((int)((int64_t)(s + 1) * G / RED_SPLIT) <= q) ++s;
@@ -1581,7 +1582,7 @@ __device__ __forceinline__ bool slice_reduce(const PassArgs& a) {
   __syncthreads();   // the CTA's partials are written
   if (threadIdx.x == 0) {
     __threadfence();
-    last = atomicInc(a.slice_cnt + s, (unsigned)(q1 - q0 - 1)) == (unsigned)(q1 - q0 - 1);
+    last = !off && atomicInc(a.slice_cnt + s, (unsigned)(q1 - q0 - 1)) == (unsigned)(q1 - q0 - 1);
     __threadfence();
   }
   __syncthreads();
