@@ -1,6 +1,7 @@
 """The Grams of the option fp64_tc above width 8 (tcgen05, exact digits) at the edges of their 64-bit frame: a
 128-row tile whose columns are constant just below a power of two, where the sum of a digit stack comes close to
-the frame's end; and the diagonal of an unconjugated Gram, sum re^2 - sum im^2, where the two nearly cancel.
+the frame's end; and the entries of an unconjugated Gram, sum re re' - sum im im', where the two nearly cancel: on the
+diagonal, and beside it where columns are correlated.
 
 Bounds: the factor xi_0 of the residual's Cholesky QR satisfies xi^H xi = R^H R; with unit-variance rows the Gram
 and its Cholesky factor are accurate to a few hundred roundings (p n-term sums, condition below 10): 1e-12 of the
@@ -85,8 +86,9 @@ def _cancelling(n, p, method, seed):
 def test_diagonal_of_an_unconjugated_gram_keeps_its_small_part(method, p):
     """X_1 = V diag(G / H): the error of G's diagonal is read off X_1 (G is small, so that all other roundings are, too:
     some 1e-16 of 0.02).  Bound 2e-15 rms over the columns: each of at most 304 CTAs rounds four differences of its
-    stacks, below 0.1, i.e. sqrt(304 * 4) * 0.1 * 2^-54 = 2e-16 rms, with a factor of ten.  Sums rounded before the
-    difference miss it by a factor of five: emulated, 1.4e-14."""
+    stacks, below 0.1, i.e. sqrt(304 * 4) * 0.1 * 2^-54 = 2e-16 rms, with a factor of ten, which also holds the rounding
+    of 1563 tiles to 2^-54 of the scales (sqrt(1563 / 12) * 2^-54 = 6e-16).  Sums rounded before the difference miss it by
+    a factor of five: emulated, 1.4e-14."""
     torch = need_gpu()
     from paper_1601_05362_gb300 import blcoc
     n = 200064
@@ -100,3 +102,60 @@ def test_diagonal_of_an_unconjugated_gram_keeps_its_small_part(method, p):
         assert h.solve(B, X, method=method, tol=0.0, maxit=1) == blcoc.BLCOC_NOT_CONVERGED
         M = (torch.sum(B.conj() * X, 0) / torch.sum(B.abs().square(), 0)).cpu().numpy()
     assert np.sqrt(np.mean(np.abs(M * H - G) ** 2)) < 2e-15
+
+
+def _gram_exact(v):
+    """v^T v of integers below 2^45 in Python integers: pieces of 15 bits, whose sums FP64 holds."""
+    w = [((v >> 30)).astype(np.float64), ((v >> 15) & 0x7FFF).astype(np.float64), (v & 0x7FFF).astype(np.float64)]
+    p = v.shape[1]
+    G = [[0] * p for _ in range(p)]
+    for a in range(3):
+        for b in range(3):
+            P = w[a].T @ w[b]
+            for i in range(p):
+                for j in range(p):
+                    G[i][j] += int(P[i, j]) << (15 * (4 - a - b))
+    return G
+
+
+def _correlated(n, p, method, seed):
+    """As _cancelling, but every column has every row, and all of them share a part u (correlation one half): now the
+    entries beside the diagonal cancel too.  Entries of 44 bits, so that a tile's sums are rounded; both Grams exact."""
+    rng = np.random.default_rng(seed)
+    m = n // 2
+    cocg = method == "cocg_rq"
+    x = rng.integers(-2**43, 2**43, (m, 1)) + rng.integers(-2**43, 2**43, (m, p))
+    d = (1 + 1e-3 * rng.standard_normal((m, 1))) / (1 if cocg else np.sqrt(2))
+    y = np.clip(np.rint(x * d), -2.0**44, 2.0**44).astype(np.int64)
+    gx, gy = _gram_exact(x), _gram_exact(y)
+    G, H = np.empty((p, p)), np.empty((p, p), np.complex128)
+    for i in range(p):
+        for j in range(p):
+            a, b = gx[i][j], gy[i][j]
+            G[i, j] = (a - (b if cocg else 2 * b)) / 2**88
+            H[i, j] = (a + b) / 2**88 if cocg else complex(a / 2**88, -2 * b / 2**88)
+    B = np.empty((n, p), np.complex128)
+    B[0::2], B[1::2] = x, (1j if cocg else 1 + 1j) * y
+    diag = np.empty(n, np.complex128)
+    diag[0::2], diag[1::2] = 1, -1 if cocg else 1j
+    return B * 2.0**-44, diag, G, H
+
+
+@pytest.mark.parametrize("p", [9, 17, 32])
+@pytest.mark.parametrize("method", ["cocg_rq", "cocr_rq"])
+def test_an_unconjugated_gram_of_correlated_columns_keeps_its_small_part(method, p):
+    """X_1 = B H^-1 G: the error of G is H M - G with M from X_1 = B M.  Bound 1e-14 rms over the entries: 1563 tiles
+    rounded to 2^-54 of the scales are 6e-16 rms, and the p x p stages, of condition p, round G (below 0.5) by
+    p * 0.5 * 2^-53, 2e-15 at p = 32: a factor of four.  Real and imaginary parts summed apart reach 50 to 100 in a CTA's
+    sums, whose rounding in three adds is 0.3 * 7e-15 * (2 * 3 * 304)^(1/2) = 9e-14."""
+    torch = need_gpu()
+    from paper_1601_05362_gb300 import blcoc
+    n = 200064
+    Bh, a, G, H = _correlated(n, p, method, seed=p)
+    with blcoc.Handle(n, np.arange(n + 1, dtype=np.int32), np.arange(n, dtype=np.int32), a) as h:
+        h.set_option("fp64_tc", 1)
+        B = to_dev(torch, Bh)
+        X = torch.zeros_like(B)
+        assert h.solve(B, X, method=method, tol=0.0, maxit=1) == blcoc.BLCOC_NOT_CONVERGED
+        M = torch.linalg.solve(B.conj().T @ B, B.conj().T @ X).cpu().numpy()
+    assert np.sqrt(np.mean(np.abs(H @ M - G) ** 2)) < 1e-14
