@@ -266,7 +266,8 @@ blcoc_status blcoc_sampled_grad(blcoc_handle h, const void* Lambda, const void* 
  *                  split each row's nonzeros (interleaved) and their partial sums are
  *                  combined in a fixed order (where p * split <= 32; otherwise 1).  0: a
  *                  timed sweep of 1 / 2 / 4 on the first solve, cached for the process per
- *                  (n, nonzeros per row, p); blcoc_solve_batched with autotune != 0 also
+ *                  (device, n, nonzeros per row, p, kernel that bundle 1 runs: it differs with
+ *                  fp64_tc, and between single and batched solves); blcoc_solve_batched with autotune != 0 also
  *                  tunes it per system.  Results are bitwise reproducible for a given
  *                  bundle.  blcoc_get_stat(h, "spmm_split") reports the bundle used.
  *                  (The product of fp64_tc above p = 8, and of FP64 single solves with
@@ -294,7 +295,8 @@ blcoc_status blcoc_set_option(blcoc_handle h, const char* key, int64_t value);
  * solve, including those inside graph replays), "graph_replays", "outer_iters"
  * (refinement steps of a mixed solve),
  * "persistent_graph" (last persistent batch: 1 graph replays, 0 direct launches, -1 none),
- * "spmm_split" (SpMM row bundle of the last solve), "qr_fallbacks" (shifted-CholQR3
+ * "spmm_split" (SpMM row bundle of the last solve), "spmm_sweeps" (timed sweeps of the
+ * bundles made for this handle so far), "qr_fallbacks" (shifted-CholQR3
  * fallbacks started in the last solve), and with the
  * "timing" option "kt_ns.<kernel>" (total device nanoseconds) and "kt_n.<kernel>"
  * (launches that did work) for <kernel> in resid, spmm_gram, spmm_plain, cocr_passA,

@@ -171,6 +171,7 @@ struct blcoc_ctx {
   int cond_ok = 0;
   cudaStream_t sbody = nullptr;   // captures the conditional node's body
   int stat_spmm_split = 0;    // row bundle of the last solve
+  int stat_spmm_sweeps = 0;   // timed sweeps of the row bundles made for this handle
   int persistent_timeout_ms = 10000;   // persistent batch: limit of one wait of the kernel
   int persistent_stall = 0;   // persistent batch, test hook: no first work item is published
   int lost_wait = 0;          // test hook: the next solve ends as if a kernel's wait had run out
@@ -958,6 +959,7 @@ blcoc_status blcoc_get_stat(blcoc_handle h, const char* key, int64_t* value) {
   if (!strcmp(key, "outer_iters")) { *value = h->outer_iters; return BLCOC_OK; }
   if (!strcmp(key, "persistent_graph")) { *value = h->stat_persistent_graph; return BLCOC_OK; }
   if (!strcmp(key, "spmm_split")) { *value = h->stat_spmm_split; return BLCOC_OK; }
+  if (!strcmp(key, "spmm_sweeps")) { *value = h->stat_spmm_sweeps; return BLCOC_OK; }
   if (!strcmp(key, "qr_fallbacks")) { *value = h->h_ctrl ? h->h_ctrl->fb_count : 0; return BLCOC_OK; }
   for (int k = 0; k < kNumKinds; ++k) {
     const std::string nm(kKindNames[k]);
@@ -1243,18 +1245,20 @@ namespace {
 
 // SpMM row-bundle autotuner: time the SpMM (it writes the handle's V and partial slots,
 // which every solve overwrites) with 1, 2 and 4 lane groups per row and keep the fastest;
-// cached per (n, nnz per row, p, FP64 or tensor-core kernel set).
+// cached per (device, n, nnz per row, p, kernel of bundle 1: FP64 or tensor-core, in two launches (single solves) or one).
 std::mutex g_spmm_mutex;
 std::map<std::string, int> g_spmm_cache;
 
 int tune_spmm_split(blcoc_ctx* h, Solver& sv, bool tc) {
-  const std::string key = std::to_string(h->n) + "/" + std::to_string((h->nnz * 10 + h->n / 2) / h->n) + "/" +
-                          std::to_string(sv.p) + "/" + (tc ? "tc" : "fp64");
+  const std::string key = std::to_string(h->dev) + "/" + std::to_string(h->n) + "/" +
+                          std::to_string((h->nnz * 10 + h->n / 2) / h->n) + "/" + std::to_string(sv.p) + "/" +
+                          (tc ? "tc" : sv.spmm_one() == sv.K->spmm_gram_two ? "fp64 two" : "fp64");
   {
     std::lock_guard<std::mutex> lock(g_spmm_mutex);
     auto it = g_spmm_cache.find(key);
     if (it != g_spmm_cache.end()) return it->second;
   }
+  h->stat_spmm_sweeps++;
   PassArgs a = sv.base();
   a.ne = tri_count(sv.p);
   a.flag = 16;   // run whatever the control block says; no T apply
