@@ -386,12 +386,15 @@ struct Solver {
       record(t.e1);
       timers->push_back(t);
     }
-    launches += pass_launches(kind);
+    launches += pass_launches(kind, flag);
     last_grid = a.grid;
   }
-  int pass_launches(int kind) const {
-    if (!spmm_applies_t() && (kind == K_COCR_A || kind == K_COCG_1 || (kind == K_COCR_C && !uexpl))) return 2;
-    return kind == K_SPMM_GRAM && (!spmm_applies_t() || (K->spmm_gram_two && spmm_fn() == K->spmm_gram_two)) ? 2 : 1;
+  // kernels a pass launches: above width 8 of the tensor-core set each Gram is one of its own
+  int pass_launches(int kind, int flag) const {
+    if (spmm_applies_t()) return kind == K_SPMM_GRAM && K->spmm_gram_two && spmm_fn() == K->spmm_gram_two ? 2 : 1;
+    if (kind == K_COCR_C) return flag & 4 ? 1 : 2;    // (explicit U: no Gram)
+    if (kind == K_RESID) return flag & 1 ? 1 : 2;     // (norms only)
+    return kind == K_COCR_A || kind == K_COCG_1 || kind == K_SPMM_GRAM ? 2 : 1;
   }
   int last_grid = 0;
   // The first-stage reduction runs inside the pass where one CTA sums a slice of its partials
@@ -654,7 +657,7 @@ struct Solver {
         if (timed) timed_begin(t, K_SPMM_GRAM);
         spmm_fn()(a, h->s);
         if (timed) timed_end(t);
-        launches += pass_launches(K_SPMM_GRAM);
+        launches += pass_launches(K_SPMM_GRAM, a.flag);
         last_grid = a.grid;
       }
       reduce(E, h->ctrl);
