@@ -77,3 +77,21 @@ def test_without_the_fallback_it_is_a_breakdown(method, p, tc):
         assert np.array_equal(got[1], want[1]) and np.array_equal(got[2], want[2]), options
     got = _run(torch, blcoc, A, B, method, base, batch=True)
     assert got[3:] == want[3:] and np.array_equal(got[1], want[1]) and np.array_equal(got[2], want[2])
+
+
+@pytest.mark.parametrize("method,after", [("cocr_rq", ["spmm_gram", "cocr_passC", "small_beta"]), ("cocg_rq", ["spmm_gram", "cocg_pass2"])])
+@pytest.mark.parametrize("graph", [0, 1])
+def test_kernel_times_leave_out_what_returned_at_once(method, after, graph):
+    """Option timing, suspended in the first of M iterations: the kernels behind that QR returned at once and are run
+    again untimed, so M - 1 of each are counted, and M of those before it."""
+    torch = need_gpu()
+    from paper_1601_05362_gb300 import blcoc
+    A, Bh = _system(323, 8, seed=8)
+    with blcoc.Handle.from_csr(A) as h:
+        h.set_option("timing", 1)
+        h.set_option("graph", graph)
+        B = to_dev(torch, Bh)
+        assert h.solve(B, torch.zeros_like(B), method=method, tol=0.0, maxit=M) == blcoc.BLCOC_NOT_CONVERGED
+        assert h.stat("qr_fallbacks") == 1
+        assert h.stat("kt_n.small_alpha") == h.stat("kt_n.small_chol") == M
+        assert [h.stat("kt_n." + k) for k in after] == [M - 1] * len(after)
