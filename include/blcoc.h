@@ -257,9 +257,10 @@ blcoc_status blcoc_sampled_grad(blcoc_handle h, const void* Lambda, const void* 
  *                  kernels from the start, as the body of a conditional node that the
  *                  Cholesky stage enables only when a fallback has started, so an iteration
  *                  that needs none launches none of them (same results bit for bit).
- *                  0 (default): the solve suspends itself, see "qr_fallback"; Nsight Compute does not profile the kernel nodes of a
- *                  graph that can hold conditional nodes.  If the runtime refuses the
- *                  conditional node the option turns itself off.  Also read per handle by
+ *                  0 (default): the solve suspends itself, see "qr_fallback"; Nsight Compute
+ *                  does not profile the kernel nodes of a graph that can hold conditional
+ *                  nodes.  If the runtime refuses the conditional node the option turns
+ *                  itself off.  Also read per handle by
  *                  blcoc_solve_batched.
  *   "spmm_split" : the SpMM's row bundle.  1 (default): p lanes per row (one per column),
  *                  each summing the row's nonzeros in order.  2 or 4: that many lane groups
@@ -286,7 +287,10 @@ blcoc_status blcoc_sampled_grad(blcoc_handle h, const void* Lambda, const void* 
  *                  the internal stream (also inside the graph) and accumulates per-kernel
  *                  device time; 2 brackets only the row-pass kernels (less overhead:
  *                  two event records per pass); 3 only the dominant row pass (pass C of
- *                  bl_cocr_rq, pass 1 of bl_cocg_rq); 0 (default) records nothing.
+ *                  bl_cocr_rq, pass 1 of bl_cocg_rq); 0 (default) records nothing.  At
+ *                  p <= 4 the timed sequence is another one (same results): the p x p
+ *                  stages, which otherwise run at the end of the passes, are kernels of
+ *                  their own, so that they can be timed.
  * Returns BLCOC_ERR_INVALID_ARG for an unknown key or value.
  */
 blcoc_status blcoc_set_option(blcoc_handle h, const char* key, int64_t value);

@@ -397,11 +397,6 @@ struct Solver {
     return kind == K_COCR_A || kind == K_COCG_1 || kind == K_SPMM_GRAM ? 2 : 1;
   }
   int last_grid = 0;
-  // The first-stage reduction runs inside the pass where one CTA sums a slice of its partials
-  // about as fast as k_reduce_stage1 spread over the GPU: a slice costs that CTA
-  // ceil(ncomp / 128) adds (about 64 clocks each) per partial: at 40 of them 1.2 us, the time the
-  // kernel's launch takes.  Solve of n = 1024, p = 4 (3 adds): 3.92 -> 3.75 ms; 16 uneven 2D
-  // systems as graph branches (up to 38): 64.7 -> 63.5 ms.  p = 16 from 64^3 on (87) keeps the kernel.
   // Widths up to 4 of the FP64 rq methods: the p x p stages run in the passes before them (pass_end), so an
   // iteration has three launches, and the alpha' step of an iteration belongs to the end of the one before.
   // n = 1024, p = 4: 2.11 -> 2.03 ms for 40 iterations; 16 uneven 2D systems as graph branches 61.7 -> 58.9 ms.
@@ -413,6 +408,11 @@ struct Solver {
     a.hist = h->hist;
   }
   int tail(PassTail t) { return next_tail = tails ? (int)t : (int)TAIL_NONE; }
+  // The first-stage reduction runs inside the pass where one CTA sums a slice of its partials
+  // about as fast as k_reduce_stage1 spread over the GPU: a slice costs that CTA
+  // ceil(ncomp / 128) adds (about 64 clocks each) per partial: at 40 of them 1.2 us, the time the
+  // kernel's launch takes.  Solve of n = 1024, p = 4 (3 adds): 3.92 -> 3.75 ms; 16 uneven 2D
+  // systems as graph branches (up to 38): 64.7 -> 63.5 ms.  p = 16 from 64^3 on (87) keeps the kernel.
   static constexpr int FUSE_MAX = 40;
   bool fused = false;
   void fuse_reduce(PassArgs& a, int kind) {

@@ -257,11 +257,6 @@ constexpr bool m3_apply() { return sizeof(S) == 8 && !OZ && PP >= 8; }
 template <int PP, typename S, bool OZ>
 constexpr bool one_tile() { return PP >= 32 && sizeof(S) == 8 && !OZ; }
 
-// Tensor-core Grams (exact slices, per-warp FP64 sums in shared memory) are built for
-// p <= 16; at p = 32 the tensor-core passes keep their Grams on the FP64 pipe (the sums
-// of 64 x 64 real entries per warp would not fit beside the tiles).
-template <int PP, bool OZ>
-constexpr bool oz_gram() { return OZ && PP <= 16; }
 // Widths above 8 of the tensor-core set: passes A, C, 1 and 2 and the SpMM's Gram are the tcgen05 kernels
 // of blcoc_tc5_pass.cuh, the SpMM's product is k_spmm_plain, and pass C applies T to it.
 template <int PP, bool OZ>
@@ -960,9 +955,9 @@ __device__ __forceinline__ void d_spmm_gram(const PassArgs& a, const int vblk, c
   BLCOC_PROLOGUE(C)
   using G = Geo<PP, S>;
   constexpr bool M3A = m3_apply<PP, S, OZ>();
-  // W for the Gram read from global memory: the FP64 SpMM at p = 32 and every tensor-core
-  // SpMM (at p <= 16 its W^T Y slices are cut from global memory, so that the tile and the
-  // per-warp Gram sums allow 3 CTAs per SM instead of 2)
+  // W for the Gram read from global memory: the FP64 SpMM at p = 32 and the tensor-core SpMM
+  // (its W^T Y slices are cut from global memory, so that the tile and the per-warp Gram
+  // sums allow 3 CTAs per SM instead of 2)
   constexpr bool OT = one_tile<PP, S, OZ>() || OZ;
   C* T_s = smem;
   C* tiles = smem + ((M3A || OZ) ? 0 : mats_off<PP, S>(1));   // the tensor-core apply reads slices
@@ -976,9 +971,8 @@ __device__ __forceinline__ void d_spmm_gram(const PassArgs& a, const int vblk, c
   Fac<PP, S> T{G::MATS_SMEM ? T_s : reinterpret_cast<const C*>(a.mats + M_TINV * PMAX * PMAX), p};
   GramAcc<G::NTRI, S> g;
   g.init(G_SYM, p, lane);
-  constexpr bool OZG = oz_gram<PP, OZ>();
   double* zsums = reinterpret_cast<double*>(tiles + NWARP * (OT ? 1 : 2) * G::TILE);   // tensor-core Gram sums
-  if constexpr (OZG) {
+  if constexpr (OZ) {
     for (int i = lane; i < OzGramGeo<PP>::ACC; i += 32) zsums[warp * OzGramGeo<PP>::ACC + i] = 0.0;
   }
   double dummy0 = 0.0, dummy1 = 0.0;
@@ -989,7 +983,7 @@ __device__ __forceinline__ void d_spmm_gram(const PassArgs& a, const int vblk, c
         tY, a.A, vals_of<S>(a.A), blk<C>(a.W), nullptr, r0, p, lane, dummy0, dummy1);
     if (!OT && !(a.flag & F_UEXPL)) load_tile<PP>(tW, blk<C>(a.W), r0, n, p, lane);   // Y^T Y needs no W
     __syncwarp();
-    if constexpr (OZG) {
+    if constexpr (OZ) {
       if (a.flag & F_UEXPL)
         oz_gram_add<PP, true>(zsums + warp * OzGramGeo<PP>::ACC, tY, tY, p, lane);
       else
@@ -1017,7 +1011,7 @@ __device__ __forceinline__ void d_spmm_gram(const PassArgs& a, const int vblk, c
     __syncwarp();
   }
   __syncthreads();
-  if constexpr (OZG) oz_gram_write<PP, false>(zsums, a.partials + (int64_t)vblk * a.ne, p, NWARP);
+  if constexpr (OZ) oz_gram_write<PP, false>(zsums, a.partials + (int64_t)vblk * a.ne, p, NWARP);
   else cta_write_gram(g, reinterpret_cast<double2*>(tiles), a.partials + (int64_t)vblk * a.ne, warp, lane);
 }
 // Two tiles per warp allow at most 3 CTAs per SM (1 at PP = 32), so registers up to that
@@ -1059,7 +1053,6 @@ __device__ __forceinline__ void d_cocr_passA(const PassArgs& a, const int vblk, 
   BLCOC_PROLOGUE(C)
   using G = Geo<PP, S>;
   constexpr bool M3A = m3_apply<PP, S, OZ>();
-  constexpr bool OZG = oz_gram<PP, OZ>();
   constexpr bool OT = one_tile<PP, S, OZ>();   // U read from global memory, four-product Gram
   // W^H W: three products where the applies take them and two tiles are kept; the tensor-core
   // pass forms it on the tensor cores
@@ -1076,7 +1069,7 @@ __device__ __forceinline__ void d_cocr_passA(const PassArgs& a, const int vblk, 
   GramAcc<G::NTRI, S, M3G> g;
   g.init(G_HERM, p, lane);
   double* zsums = reinterpret_cast<double*>(tiles + NWARP * 2 * G::TILE);   // tensor-core Gram sums
-  if constexpr (OZG) {
+  if constexpr (OZ) {
     for (int i = lane; i < OzGramGeo<PP>::ACC; i += 32) zsums[warp * OzGramGeo<PP>::ACC + i] = 0.0;
   }
   for (int64_t c = (int64_t)vblk * NWARP + warp; c < nchunks; c += cstride) {
@@ -1097,14 +1090,14 @@ __device__ __forceinline__ void d_cocr_passA(const PassArgs& a, const int vblk, 
       apply_full<PP, S, true>(tW, tW, tU, AL, p, lane);    // W_{m+1} = Q_m - U_m alpha'
     }
     __syncwarp();
-    if constexpr (OZG) oz_gram_add<PP, true>(zsums + warp * OzGramGeo<PP>::ACC, tW, tW, p, lane);
+    if constexpr (OZ) oz_gram_add<PP, true>(zsums + warp * OzGramGeo<PP>::ACC, tW, tW, p, lane);
     else if constexpr (M3G) g.template add3<true>(tW, tU, lane);
     else g.template add<true>(tW, tW, lane);
     store_tile<PP>(blk<C>(a.W), tW, r0, n, p, lane);
     __syncwarp();
   }
   __syncthreads();
-  if constexpr (OZG) oz_gram_write<PP, true>(zsums, a.partials + (int64_t)vblk * a.ne, p, NWARP);
+  if constexpr (OZ) oz_gram_write<PP, true>(zsums, a.partials + (int64_t)vblk * a.ne, p, NWARP);
   else cta_write_gram(g, reinterpret_cast<double2*>(tiles), a.partials + (int64_t)vblk * a.ne, warp, lane);
 }
 // FP64: two tiles per warp allow at most 3 CTAs per SM (1 at PP = 32), so registers up to
@@ -1689,7 +1682,7 @@ constexpr size_t pass_smem(int kind) {
   const bool has_gram =
       kind == K_SPMM_GRAM || kind == K_COCR_A || kind == K_COCR_C || kind == K_COCG_1 || kind == K_QR2;
   if (has_gram && s < mats + red) s = mats + red;
-  if (oz_gram<PP, OZ>() && (kind == K_COCR_A || kind == K_SPMM_GRAM))
+  if (OZ && (kind == K_COCR_A || kind == K_SPMM_GRAM))
     s += (size_t)NWARP * OzGramGeo<PP>::ACC * sizeof(double);
   return s;
 }
