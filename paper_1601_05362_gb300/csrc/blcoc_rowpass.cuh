@@ -830,6 +830,7 @@ constexpr bool narrow() { return PP <= 4 && sizeof(S) == 8; }
 #include "blcoc_small_w4.cuh"
 namespace blcoc {
 
+template <bool T5 = false>
 __device__ __forceinline__ bool slice_reduce(const PassArgs& a);
 template <int PP, typename S>
 __device__ __forceinline__ void pass_end(const PassArgs& a);
@@ -1562,12 +1563,16 @@ __global__ void __launch_bounds__(256) k_axpy(const PassArgs a) {
 // so the sums are the same bits.  Saves that kernel's launch (about 3.5 us of a 2D iteration)
 // where one CTA can sum a slice as quickly: see Solver::fuse_reduce for the line.
 // Returns whether this CTA summed the last slice of all (with a.tail; its slices are then all written).
+// T5: a tcgen05 kernel, where a CTA that gave up a wait sets `done` while others are here: one read for the CTA.
+// (Elsewhere every thread reads it and leaves at once: a launch past the end then runs no barrier and no fence,
+// 32^2, p = 4 2063 -> 2045 us.)
+template <bool T5>
 __device__ __forceinline__ bool slice_reduce(const PassArgs& a) {
   if (a.slice_cnt == nullptr) return false;
   __shared__ int last;
-  // one read for the CTA: a tcgen05 kernel's CTA that gave up a wait sets `done` while others are here
-  const bool off = threadIdx.x == 0 && ((!(a.flag & F_FORCE) && BLCOC_LD(&a.ctrl->done)) ||
-                                        ((a.flag & F_FB) && BLCOC_LD(&a.ctrl->qr_fb) == 0));
+  const bool off = (!T5 || threadIdx.x == 0) && ((!(a.flag & F_FORCE) && BLCOC_LD(&a.ctrl->done)) ||
+                                                 ((a.flag & F_FB) && BLCOC_LD(&a.ctrl->qr_fb) == 0));
+  if (!T5 && off) return false;
   const int G = gridDim.x, q = blockIdx.x;
   int s = (int)((int64_t)q * RED_SPLIT / G);
   while ((int)((int64_t)(s + 1) * G / RED_SPLIT) <= q) ++s;
