@@ -229,7 +229,8 @@ blcoc_status blcoc_sampled_grad(blcoc_handle h, const void* Lambda, const void* 
  *                  row passes' Grams with it; p <= 8 with warp-level instructions (eight
  *                  7-bit digits in bf16, 43 products), and for BLCOC_COCR_RQ the Grams
  *                  W^H W and W^T A W.  The other Grams, the sparse product and the p x p
- *                  stages stay FP64.  0 (default) computes everything with FP64 FMAs
+ *                  stages stay FP64.  Accuracy is relative to the largest entry of a row:
+ *                  scale columns of B of very different size.  0 (default) computes everything with FP64 FMAs
  *                  (so do p <= 4, the plain methods and the complex64 inner solves).
  *   "u_explicit_mixed": the same for the complex64 inner solves of BLCOC_COCR_RQ_MIXED
  *                  (default 1: the recurrence drifts quickly in single precision).
